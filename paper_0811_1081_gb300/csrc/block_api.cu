@@ -167,8 +167,7 @@ extern "C" gspca_status gspca_fit_block(gspca_t h, void* stream, const float* X,
     int launches = 0;
     const int center = opts ? opts->center : 0;
     if (center == 1) {
-        colmean_kernel<<<(N + 7) / 8, 256, 0, s>>>(X, (int)layout, ldx, M, N, h->ws.cmean);
-        ++launches;
+        launches += enqueue_colmean(h->ws, s, X, layout, ldx, M, N);
     } else if (center == 2) {
         rowmean_kernel<<<(M + 7) / 8, 256, 0, s>>>(X, (int)layout, ldx, M, N, h->ws.rmean);
         ++launches;

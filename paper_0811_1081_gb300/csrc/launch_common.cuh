@@ -295,6 +295,28 @@ inline FitArgs make_args(const Workspace& w, const Plan& p, int M, int N, int K,
     return a;
 }
 
+// Column means of X into w.cmean; the chunk sums go where the fit's pass partials will
+// (w.G x w.LA floats).  Returns the kernels launched.
+inline int enqueue_colmean(const Workspace& w, cudaStream_t s, const float* X, gspca_layout layout, long ldx, int M,
+                           int N) {
+    const int gx = (N + 31) / 32;
+    const size_t room = sizeof(float) * (size_t)w.G * w.LA / (sizeof(double) * (size_t)N);
+    int chunks = (608 + gx - 1) / gx;  // four blocks per SM
+    if (chunks > 64) chunks = 64;
+    if ((size_t)chunks > room) chunks = (int)room;
+    if (chunks < 2) {
+        colmean_kernel<<<(N + 7) / 8, 256, 0, s>>>(X, (int)layout, ldx, M, N, w.cmean);
+        return 1;
+    }
+    int rows_per = (M + chunks - 1) / chunks;
+    if (rows_per < 64) rows_per = 64;
+    chunks = (M + rows_per - 1) / rows_per;
+    double* part = reinterpret_cast<double*>(w.partA);
+    colmean_part_kernel<<<dim3(gx, chunks), 256, 0, s>>>(X, (int)layout, ldx, M, N, rows_per, part);
+    colmean_sum_kernel<<<(N + 127) / 128, 128, 0, s>>>(part, chunks, M, N, w.cmean);
+    return 2;
+}
+
 // Enqueue the launch sequence of one fit on `s` (no synchronisation).
 // Returns the number of kernels enqueued through *launches.
 inline cudaError_t enqueue_sequence(const Workspace& w, const Plan& p, FitArgs a, cudaStream_t s, const float* X,
@@ -304,8 +326,7 @@ inline cudaError_t enqueue_sequence(const Workspace& w, const Plan& p, FitArgs a
     const int M = a.M, N = a.N, K = a.K, np = a.np;
     int n = 0;
     if (center == 1) {
-        colmean_kernel<<<(N + 7) / 8, 256, 0, s>>>(X, (int)layout, ldx, M, N, w.cmean);
-        ++n;
+        n += enqueue_colmean(w, s, X, layout, ldx, M, N);
     } else if (center == 2) {
         rowmean_kernel<<<(M + 7) / 8, 256, 0, s>>>(X, (int)layout, ldx, M, N, w.rmean);
         ++n;
