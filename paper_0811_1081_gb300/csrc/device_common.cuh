@@ -284,6 +284,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return done != 0;
 }
 
+// A ring wait that gave up after the caller's limit is reported as a timeout,
+// but the copy it waited for was issued and normally lands a little later: the
+// stage is awaited again, for at most this long, before it is read, refilled
+// or abandoned, so that no copy is still in flight when its stage (or the
+// CTA's shared memory) is reused.
+constexpr unsigned long long kSettleNs = 1000000000ull;
+
 // Bounded wait for phase `parity` of `bar`; false after `timeout_ns`.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t timeout_ns) {
     if (mbar_try_wait(bar, parity)) return true;

@@ -44,7 +44,7 @@ __global__ void rowmean64_kernel(const double* X, int layout, long ldx, int M, i
 // ||R||_F^2 partial per block (fixed grid, so the sum has a fixed order).  Block
 // 0 also clears the barrier counter, the abort words and the info words.
 __global__ void __launch_bounds__(256) pack64_kernel(const double* X, int layout, long ldx, int M, int N, int center,
-                                                     const double* cmean, const double* rmean, double* R,
+                                                     const double* cmean, const double* rmean, double* R, int ldr,
                                                      double* xpart, unsigned* flags, int* abort, int* info) {
     __shared__ double red[8];
     const int t = threadIdx.x;
@@ -68,7 +68,8 @@ __global__ void __launch_bounds__(256) pack64_kernel(const double* X, int layout
         double v = load_x64(X, layout, ldx, r, c);
         if (center == 1) v -= cmean[c];
         else if (center == 2) v -= rmean[r];
-        R[(size_t)r * N + c] = v;
+        R[(size_t)r * ldr + c] = v;
+        if (ldr > N && c == N - 1) R[(size_t)r * ldr + N] = 0.0;
         sq = fma(v, v, sq);
     }
     sq = warp_sum(sq);
@@ -112,33 +113,41 @@ __global__ void epilogue64_kernel(const double* V, const double* U, int ld, cons
 // R_out (M x N, ld M) from the row-major residual; when every component was found,
 // the deflation of the last one (Eq. 3) is applied here, as the fit applies it
 // inside the next component's first sweep.
-__global__ void unpack64_kernel(const double* R, const double* V, const double* U, int ld, const double* lam_ws,
+__global__ void unpack64_kernel(const double* R, int ldr, const double* V, const double* U, int ld, const double* lam_ws,
                                 const int* info, int M, int N, int K, int gs, double* Rout) {
     const bool defl = info[1] == K;
     const double lamf = gs ? lam_ws[K - 1] : 1.0;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < (size_t)M * N; i += stride) {
         const int r = (int)(i % M), c = (int)(i / M);
-        double v = R[(size_t)r * N + c];
+        double v = R[(size_t)r * ldr + c];
         if (defl) v = fma(-lamf * V[(size_t)r * ld + (K - 1)], U[(size_t)c * ld + (K - 1)], v);
         Rout[i] = v;
     }
 }
 
-// Rows per staged chunk and dynamic shared memory for N columns; rc = 0 when
-// even one row does not fit.
-cudaError_t plan64(int device, int N, int ldk, int G, int* rc, size_t* dyn) {
+// Rows per staged chunk, chunks in shared memory and its bytes for rows of ldr doubles;
+// rc = 0 when even one row does not fit.  Three chunks (the sweep's pipeline) of four, two
+// or one rows where they fit (ldr up to about 2000, 3500, 5600), else one chunk of as many
+// rows as fit.
+cudaError_t plan64(int device, int ldr, int N, int ldk, int G, int* rc, int* nbuf, size_t* dyn) {
     int optin = 0;
     cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     if (e != cudaSuccess) return e;
     cudaFuncAttributes fa{};
     if ((e = cudaFuncGetAttributes(&fa, fit64_kernel)) != cudaSuccess) return e;
     const int max_slice = (N + G - 1) / G + 1;
-    const long avail = (long)optin - (long)fa.sharedSizeBytes - 1024;
-    int r = 0;
-    while (r < kMaxRc64 && (long)smem64_bytes(N, r + 1, ldk, max_slice) <= avail) ++r;
-    *rc = r;
-    *dyn = smem64_bytes(N, r > 0 ? r : 1, ldk, max_slice);
+    const long avail = (long)optin - (long)fa.sharedSizeBytes - 256;
+    *rc = 0;
+    *nbuf = 1;
+    for (int r : {4, 2, 1})
+        if (*rc == 0 && (long)smem64_bytes(ldr, 3, r, ldk, max_slice) <= avail) {
+            *rc = r;
+            *nbuf = 3;
+        }
+    for (int r : {4, 3, 2, 1})
+        if (*rc == 0 && (long)smem64_bytes(ldr, 1, r, ldk, max_slice) <= avail) *rc = r;
+    *dyn = smem64_bytes(ldr, *nbuf, *rc > 0 ? *rc : 1, ldk, max_slice);
     return cudaSuccess;
 }
 
@@ -183,9 +192,10 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
     int G = h->num_sms < M ? h->num_sms : M;
     if (opts && opts->grid_ctas > 0 && opts->grid_ctas < G) G = opts->grid_ctas;
     const int ldk = w.ld;
-    int rc = 0;
+    const int ldr = (N + 1) / 2 * 2;
+    int rc = 0, nbuf = 1;
     size_t dyn = 0;
-    GS_CUDA(plan64(h->device, N, ldk, G, &rc, &dyn));
+    GS_CUDA(plan64(h->device, ldr, N, ldk, G, &rc, &nbuf, &dyn));
     if (rc < 1) return GSPCA_ERR_NOT_SUPPORTED;
     GS_CUDA(cudaFuncSetAttribute(fit64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
     int bps = 0;
@@ -207,8 +217,8 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
         rowmean64_kernel<<<(M + 7) / 8, 256, 0, s>>>(X, (int)layout, ldx, M, N, w.rmean);
         ++launches;
     }
-    pack64_kernel<<<kPack64Blocks, 256, 0, s>>>(X, (int)layout, ldx, M, N, center, w.cmean, w.rmean, w.R, w.xpart,
-                                                w.flags, w.abort, w.info);
+    pack64_kernel<<<kPack64Blocks, 256, 0, s>>>(X, (int)layout, ldx, M, N, center, w.cmean, w.rmean, w.R, ldr,
+                                                w.xpart, w.flags, w.abort, w.info);
     ++launches;
     GS_CUDA(cudaGetLastError());
 
@@ -228,7 +238,6 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
     a.W = w.W;
     a.ldk = ldk;
     a.vraw = w.vraw;
-    a.vcorr = w.vcorr;
     a.ut = w.ut;
     a.upre = w.upre;
     a.partS = w.partS;
@@ -243,6 +252,8 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
     a.iters_lock = lock_dev;
     a.timeout_ns = (unsigned long long)(timeout * 1e9);
     a.rc = rc;
+    a.nbuf = nbuf;
+    a.ldr = ldr;
     void* args[] = {&a};
     GS_CUDA(cudaEventRecord(h->ev0, s));
     GS_CUDA(cudaLaunchCooperativeKernel((const void*)fit64_kernel, dim3(G), dim3(kBlock64), args, dyn, s));
@@ -252,7 +263,8 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
                                           (opts && opts->svd_form == 1) ? 1 : 0, T, P, lambda, iters);
     ++launches;
     if (R_out) {
-        unpack64_kernel<<<1024, 256, 0, s>>>(w.R, w.V, w.U, ldk, w.lam, w.info, M, N, K, algo == GSPCA_GS, R_out);
+        unpack64_kernel<<<1024, 256, 0, s>>>(w.R, ldr, w.V, w.U, ldk, w.lam, w.info, M, N, K,
+                                              algo == GSPCA_GS, R_out);
         ++launches;
     }
     GS_CUDA(cudaGetLastError());

@@ -211,13 +211,6 @@ __device__ __forceinline__ void ring_prefetch(const FitArgs& f, Ring& rg, int p0
     for (int i = (int)(rg.issued - rg.used); i < rg.S && i < nrounds; ++i) ring_issue<E>(f, rg, p0, p1, ppr, i);
 }
 
-// A ring wait that gave up after the caller's limit is reported as a timeout,
-// but the copy it waited for was issued and normally lands a little later: the
-// stage is awaited again, for at most this long, before it is read, refilled
-// or abandoned, so that no copy is still in flight when its stage (or the
-// CTA's shared memory) is reused.
-constexpr unsigned long long kSettleNs = 1000000000ull;
-
 // Testing hook: wait, bounded by the caller's limit, for a word that nothing
 // sets; returns false when the limit runs out.
 __device__ __forceinline__ bool stall_wait(const FitArgs& f) {

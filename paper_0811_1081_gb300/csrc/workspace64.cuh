@@ -10,7 +10,7 @@ namespace gspca {
 constexpr int kPack64Blocks = 2048;  // pack kernel grid: one ||X||_F^2 partial per block
 
 struct Workspace64 {
-    double *R, *V, *U, *W, *vraw, *vcorr, *ut, *upre, *partS, *partA, *scal, *lam, *xpart, *cmean, *rmean;
+    double *R, *V, *U, *W, *vraw, *ut, *upre, *partS, *partA, *scal, *lam, *xpart, *cmean, *rmean;
     int *iters, *info, *abort, *lock;
     unsigned* flags;
     int ld, LS, G;
@@ -33,12 +33,11 @@ inline Workspace64 carve64_ws(void* base, long M, int N, int K, int G) {
         off += (bytes > 0 ? bytes : 1);
         return p;
     };
-    w.R = (double*)take(sizeof(double) * (size_t)M * N);
+    w.R = (double*)take(sizeof(double) * (size_t)M * ((N + 1) / 2 * 2));  // rows padded to 16 bytes
     w.V = (double*)take(sizeof(double) * (size_t)M * w.ld);
     w.U = (double*)take(sizeof(double) * (size_t)N * w.ld);
     w.W = (double*)take(sizeof(double) * (size_t)N * w.ld);
     w.vraw = (double*)take(sizeof(double) * (size_t)M);
-    w.vcorr = (double*)take(sizeof(double) * (size_t)M);
     w.ut = (double*)take(sizeof(double) * 2 * (size_t)N);
     w.upre = (double*)take(sizeof(double) * (size_t)N);
     w.partS = (double*)take(sizeof(double) * (size_t)G * w.LS);
