@@ -10,11 +10,12 @@
 // with the Gram matrix accumulated in FP64 (block_kernels.cuh).  The residual
 // lives column-major in the handle's R buffer; V and U are kept in the caller's
 // T and P (unit columns until the block ends).  One host synchronisation per
-// iteration reads the stop and degenerate flags.
+// iteration reads the stop and degenerate flags, behind the next half step.
 #include <cublas_v2.h>
 #include <cuda_runtime.h>
 
 #include <cstring>
+#include <utility>
 #include <vector>
 
 #include "../../include/gspca.h"
@@ -35,8 +36,8 @@ namespace {
     } while (0)
 
 struct BlockWs {
-    float *Y, *V, *Z, *U, *tmp, *Sinv, *Yh, *Zh;
-    double *part, *G, *Bm, *ev, *evec, *sp, *sigma;
+    float *Y, *V, *Vnext, *Z, *U, *Unext, *tmp, *Sinv, *Yh, *Zh;
+    double *part, *partZ, *sp, *sigma;
     int* flag;
     size_t bytes;
 };
@@ -54,17 +55,16 @@ BlockWs carve_block(void* base, long M, int N, int K) {
     const size_t B = kBlkMax;
     w.Y = (float*)take(sizeof(float) * (size_t)M * B);
     w.V = (float*)take(sizeof(float) * (size_t)M * B);
+    w.Vnext = (float*)take(sizeof(float) * (size_t)M * B);
     w.Z = (float*)take(sizeof(float) * (size_t)N * B);
     w.U = (float*)take(sizeof(float) * (size_t)N * B);
+    w.Unext = (float*)take(sizeof(float) * (size_t)N * B);
     w.tmp = (float*)take(sizeof(float) * (size_t)((size_t)K > B ? (size_t)K : B) * B);
     w.Sinv = (float*)take(sizeof(float) * B * B);
     w.Yh = (float*)take(sizeof(float) * B * B);
     w.Zh = (float*)take(sizeof(float) * B * B);
-    w.part = (double*)take(sizeof(double) * kGramCtas * B * B);
-    w.G = (double*)take(sizeof(double) * B * B);
-    w.Bm = (double*)take(sizeof(double) * B * B);
-    w.ev = (double*)take(sizeof(double) * B);
-    w.evec = (double*)take(sizeof(double) * B * B);
+    w.part = (double*)take(sizeof(double) * kGramParts * B * B);
+    w.partZ = (double*)take(sizeof(double) * kGramParts * B * B);
     w.sp = (double*)take(sizeof(double) * B);
     w.sigma = (double*)take(sizeof(double) * B);
     w.flag = (int*)take(sizeof(int) * 4);
@@ -72,31 +72,29 @@ BlockWs carve_block(void* base, long M, int N, int K) {
     return w;
 }
 
-// Gram matrix out = A^T B (n x m, FP64) of FP32 column-major A (rows x n), B (rows x m).
-void gram(cudaStream_t s, const float* A, int lda, const float* B, int ldb, int rows, int n, int m, const BlockWs& w,
-          double* out) {
-    gram_part_kernel<<<kGramCtas, 1024, 0, s>>>(A, lda, B, ldb, rows, n, m, w.part);
-    gram_sum_kernel<<<1, 1024, 0, s>>>(w.part, kGramCtas, n, m, out);
+// Gram matrix A^T B (n x m, FP64) of FP32 column-major A (rows x n), B (rows x m), as
+// kGramParts parts.
+void gram(cudaStream_t s, const float* A, int lda, const float* B, int ldb, int rows, int n, int m, double* part) {
+    gram_part_kernel<<<kGramCtas, kGramThreads, 0, s>>>(A, lda, B, ldb, rows, n, m, part);
 }
 
 // Cholesky QR applied twice: Q (rows x n) = A S1^{-1} S2^{-1}, A left unchanged
-// unless Q == A is not required (Q and A distinct buffers).  `have_gram`: w.G
-// already holds A^T A.
+// (Q and A distinct buffers).  `have`: the parts of A^T A where they are formed already.
 gspca_status cholqr2(cublasHandle_t cb, cudaStream_t s, const float* A, float* Q, int rows, int n, const BlockWs& w,
-                     bool have_gram, int* launches) {
+                     const double* have, int* flag, int* launches) {
     const float one = 1.f, zero = 0.f;
-    if (!have_gram) {
-        gram(s, A, rows, A, rows, rows, n, n, w, w.G);
-        *launches += 2;
+    if (!have) {
+        gram(s, A, rows, A, rows, rows, n, n, w.part);
+        ++*launches;
     }
-    chol_inv_kernel<<<1, 256, 0, s>>>(w.G, n, w.Sinv, w.flag);
+    chol_inv_kernel<<<1, 128, 0, s>>>(have ? have : w.part, n, w.Sinv, flag);
     BL_CUBLAS(cublasSgemm(cb, CUBLAS_OP_N, CUBLAS_OP_N, rows, n, n, &one, A, rows, w.Sinv, n, &zero, Q, rows));
-    gram(s, Q, rows, Q, rows, rows, n, n, w, w.G);
-    chol_inv_kernel<<<1, 256, 0, s>>>(w.G, n, w.Sinv, w.flag);
+    gram(s, Q, rows, Q, rows, rows, n, n, w.part);
+    chol_inv_kernel<<<1, 128, 0, s>>>(w.part, n, w.Sinv, flag);
     // Q <- Q S2^{-1} in place: an upper-triangular factor on the right (column j uses columns <= j)
     BL_CUBLAS(cublasStrmm(cb, CUBLAS_SIDE_RIGHT, CUBLAS_FILL_MODE_UPPER, CUBLAS_OP_N, CUBLAS_DIAG_NON_UNIT, rows, n,
                           &one, w.Sinv, n, Q, rows, Q, rows));
-    *launches += 6;
+    *launches += 5;
     return GSPCA_OK;
 }
 
@@ -116,6 +114,11 @@ gspca_status gspca::block_release(gspca_handle* h) {
     if (h->blk_base && cudaFree(h->blk_base) != cudaSuccess) st = GSPCA_ERR_CUDA;
     if (h->cublas) cublasDestroy((cublasHandle_t)h->cublas);
     if (h->h_blk) cudaFreeHost(h->h_blk);
+    if (h->blk_stream) cudaStreamDestroy(h->blk_stream);
+    if (h->blk_gram) cudaEventDestroy(h->blk_gram);
+    if (h->blk_test) cudaEventDestroy(h->blk_test);
+    h->blk_stream = nullptr;
+    h->blk_gram = h->blk_test = nullptr;
     h->blk_base = nullptr;
     h->cublas = nullptr;
     h->h_blk = nullptr;
@@ -153,12 +156,20 @@ extern "C" gspca_status gspca_fit_block(gspca_t h, void* stream, const float* X,
             return GSPCA_ERR_CUDA;
         }
         h->cublas = cb;
+        int lo = 0, hi = 0;
+        if (!cuda_ok(cudaDeviceGetStreamPriorityRange(&lo, &hi)) ||
+            !cuda_ok(cudaStreamCreateWithPriority(&h->blk_stream, cudaStreamNonBlocking, hi)) ||
+            !cuda_ok(cudaEventCreateWithFlags(&h->blk_gram, cudaEventDisableTiming)) ||
+            !cuda_ok(cudaEventCreateWithFlags(&h->blk_test, cudaEventDisableTiming))) {
+            block_release(h);
+            return GSPCA_ERR_CUDA;
+        }
         if (!cuda_ok(cudaMallocHost((void**)&h->h_blk, sizeof(int) * 4))) {
             block_release(h);
             return GSPCA_ERR_CUDA;
         }
     }
-    const BlockWs w = carve_block(h->blk_base, h->max_M, (int)h->max_N, h->max_K);
+    BlockWs w = carve_block(h->blk_base, h->max_M, (int)h->max_N, h->max_K);
     cublasHandle_t cb = (cublasHandle_t)h->cublas;
     BL_CUBLAS(cublasSetStream(cb, s));
     BL_CUBLAS(cublasSetMathMode(cb, CUBLAS_DEFAULT_MATH));  // FP32 products, no TF32
@@ -188,51 +199,63 @@ extern "C" gspca_status gspca_fit_block(gspca_t h, void* stream, const float* X,
         // U = R^T R(:, k0 .. k0+bw-1), against U_(k0), orthonormal
         BL_CUBLAS(cublasSgemm(cb, CUBLAS_OP_T, CUBLAS_OP_N, N, bw, M, &one, R, M, R + (size_t)k0 * M, M, &zero, w.Z, N));
         if (project_out(cb, P, N, k0, w.Z, bw, w.tmp) != GSPCA_OK) return GSPCA_ERR_CUDA;
-        if (cholqr2(cb, s, w.Z, w.U, N, bw, w, false, &launches) != GSPCA_OK) return GSPCA_ERR_CUDA;
-        int j = 0, fl = 0;
-        for (;;) {
-            // Y = R U, against V_(k0), orthonormal -> V
-            BL_CUBLAS(cublasSgemm(cb, CUBLAS_OP_N, CUBLAS_OP_N, M, bw, N, &one, R, M, w.U, N, &zero, w.Y, M));
+        if (cholqr2(cb, s, w.Z, w.U, N, bw, w, nullptr, w.flag, &launches) != GSPCA_OK) return GSPCA_ERR_CUDA;
+        // V = qr(R U), against V_(k0); `flag` takes what the factorisations find
+        auto half_step = [&](const float* U, float* V, int* flag) -> gspca_status {
+            BL_CUBLAS(cublasSgemm(cb, CUBLAS_OP_N, CUBLAS_OP_N, M, bw, N, &one, R, M, U, N, &zero, w.Y, M));
             if (project_out(cb, T, M, k0, w.Y, bw, w.tmp) != GSPCA_OK) return GSPCA_ERR_CUDA;
-            if (cholqr2(cb, s, w.Y, w.V, M, bw, w, false, &launches) != GSPCA_OK) return GSPCA_ERR_CUDA;
+            launches += 1 + (k0 > 0 ? 2 : 0);
+            return cholqr2(cb, s, w.Y, V, M, bw, w, nullptr, flag, &launches);
+        };
+        if (half_step(w.U, w.V, w.flag) != GSPCA_OK) return GSPCA_ERR_CUDA;
+        int j = 0, fl = 0;
+        bool last = false;
+        for (;;) {
             // Z = R^T V, against U_(k0); Ritz values from Z^T Z
             BL_CUBLAS(cublasSgemm(cb, CUBLAS_OP_T, CUBLAS_OP_N, N, bw, M, &one, R, M, w.V, M, &zero, w.Z, N));
             if (project_out(cb, P, N, k0, w.Z, bw, w.tmp) != GSPCA_OK) return GSPCA_ERR_CUDA;
-            gram(s, w.Z, N, w.Z, N, N, bw, bw, w, w.G);
-            jacobi_eig_kernel<<<1, 256, 0, s>>>(w.G, bw, w.ev, w.evec);
-            ritz_test_kernel<<<1, 1, 0, s>>>(w.ev, w.sp, bw, tol, w.flag);
-            launches += 6 + (k0 > 0 ? 4 : 0);
+            gram(s, w.Z, N, w.Z, N, N, bw, bw, w.partZ);
+            // The test, one CTA and a long chain, runs on a stream of its own.  The next U = qr(Z) and
+            // V = qr(R U) go ahead meanwhile, into second buffers and with the other flag word, and
+            // are dropped when the test says stop: 10000 x 2000, two blocks of 16, 6 iterations each,
+            // 6.1 ms with the test before them, 4.8 so.  Not where this iteration is the last in any
+            // case.
+            GS_CUDA(cudaEventRecord(h->blk_gram, s));
+            GS_CUDA(cudaStreamWaitEvent(h->blk_stream, h->blk_gram, 0));
+            ritz_test_kernel<<<1, kJacobiThreads, 0, h->blk_stream>>>(w.partZ, w.sp, bw, tol, w.flag + (j & 1), h->h_blk);
+            GS_CUDA(cudaGetLastError());
+            GS_CUDA(cudaEventRecord(h->blk_test, h->blk_stream));
+            launches += 3 + (k0 > 0 ? 2 : 0);
             ++j;
             ++total;
-            GS_CUDA(cudaMemcpyAsync(h->h_blk, w.flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-            GS_CUDA(cudaStreamSynchronize(s));
-            fl = h->h_blk[0];
-            if (fl & 1) break;  // dependent columns
-            bool stop;
-            if (opts && opts->iters_lock) {
-                stop = j >= opts->iters_lock[k0];
-            } else {
-                stop = (fl & 2) != 0;
-                if (!stop && j >= max_iter) {
-                    stop = true;
-                    not_converged = true;
-                }
-            }
-            if (stop) break;
-            GS_CUDA(cudaMemsetAsync(w.flag, 0, sizeof(int), s));
-            // U = qr(Z), the Gram matrix Z^T Z is already in w.G
-            if (cholqr2(cb, s, w.Z, w.U, N, bw, w, true, &launches) != GSPCA_OK) return GSPCA_ERR_CUDA;
+            last = opts && opts->iters_lock ? j >= opts->iters_lock[k0] : j >= max_iter;
+            if (last) break;
+            int* nflag = w.flag + (j & 1);
+            if (cholqr2(cb, s, w.Z, w.Unext, N, bw, w, w.partZ, nflag, &launches) != GSPCA_OK) return GSPCA_ERR_CUDA;
+            if (half_step(w.Unext, w.Vnext, nflag) != GSPCA_OK) return GSPCA_ERR_CUDA;
+            GS_CUDA(cudaEventSynchronize(h->blk_test));
+            fl = ((volatile int*)h->h_blk)[0];
+            if ((fl & 1) || (!(opts && opts->iters_lock) && (fl & 2))) break;  // dependent columns, or stop
+            std::swap(w.U, w.Unext);
+            std::swap(w.V, w.Vnext);
         }
-        if (fl & 1) {
+        if (!last && (fl & 1)) {
             status = GSPCA_ERR_DEGENERATE;
             break;
         }
         // Rayleigh-Ritz: B = Z^T U (FP64), B^T B = Zh diag(sigma^2) Zh^T, Yh = B Zh / sigma
-        gram(s, w.Z, N, w.U, N, N, bw, bw, w, w.Bm);
-        btb_kernel<<<1, 1024, 0, s>>>(w.Bm, bw, w.G);
-        jacobi_eig_kernel<<<1, 256, 0, s>>>(w.G, bw, w.ev, w.evec);
-        ritz_rot_kernel<<<1, 1024, 0, s>>>(w.Bm, w.ev, w.evec, bw, w.sigma, w.Yh, w.Zh, w.flag);
-        launches += 5;
+        gram(s, w.Z, N, w.U, N, N, bw, bw, w.part);
+        ritz_rot_kernel<<<1, kJacobiThreads, 0, s>>>(w.part, bw, w.sigma, lambda + k0, w.Yh, w.Zh, h->h_blk + 1);
+        launches += 2;
+        if (last) {
+            GS_CUDA(cudaEventSynchronize(h->blk_test));
+            fl = ((volatile int*)h->h_blk)[0];
+            if (fl & 1) {
+                status = GSPCA_ERR_DEGENERATE;
+                break;
+            }
+            if (!(opts && opts->iters_lock) && !(fl & 2)) not_converged = true;
+        }
         // V <- V Yh (into T's columns), U <- U Zh (into P's columns)
         BL_CUBLAS(cublasSgemm(cb, CUBLAS_OP_N, CUBLAS_OP_N, M, bw, bw, &one, w.V, M, w.Yh, bw, &zero,
                               T + (size_t)k0 * M, M));
@@ -241,18 +264,14 @@ extern "C" gspca_status gspca_fit_block(gspca_t h, void* stream, const float* X,
         // R -= (V diag(sigma)) U^T
         scale_cols_kernel<<<256, 256, 0, s>>>(T + (size_t)k0 * M, M, w.Y, M, M, bw, w.sigma);
         BL_CUBLAS(cublasSgemm(cb, CUBLAS_OP_N, CUBLAS_OP_T, M, N, bw, &mone, w.Y, M, P + (size_t)k0 * N, N, &one, R, M));
-        GS_CUDA(cudaMemcpyAsync(lambda + k0, w.sigma, sizeof(double) * bw, cudaMemcpyDeviceToDevice, s));
-        GS_CUDA(cudaMemcpyAsync(h->h_blk, w.flag, sizeof(int), cudaMemcpyDeviceToHost, s));
         GS_CUDA(cudaStreamSynchronize(s));
-        if (h->h_blk[0] & 1) {
+        if (((volatile int*)h->h_blk)[1] & 1) {
             status = GSPCA_ERR_DEGENERATE;
             break;
         }
         if (iters) {
-            int hi[kBlkMax];
-            for (int i = 0; i < bw; ++i) hi[i] = j;
-            GS_CUDA(cudaMemcpyAsync(iters + k0, hi, sizeof(int) * bw, cudaMemcpyHostToDevice, s));
-            GS_CUDA(cudaStreamSynchronize(s));
+            fill_int_kernel<<<1, kBlkMax, 0, s>>>(iters + k0, bw, j);
+            ++launches;
         }
         found = k0 + bw;
         blk_iters.push_back(j);

@@ -82,5 +82,7 @@ struct gspca_handle {
     gspca::Workspace64 ws64{};
     void* blk_base = nullptr;       // gspca_fit_block: block workspace (allocated on first use)
     void* cublas = nullptr;         // its cuBLAS handle
-    int* h_blk = nullptr;           // pinned flag word
+    int* h_blk = nullptr;           // pinned flag words
+    cudaStream_t blk_stream = nullptr;  // the block fit's convergence test
+    cudaEvent_t blk_gram = nullptr, blk_test = nullptr;  // its input is formed; it is done
 };
