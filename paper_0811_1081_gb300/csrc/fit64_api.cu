@@ -137,7 +137,7 @@ cudaError_t plan64(int device, int ldr, int N, int ldk, int G, int* rc, int* nbu
     cudaFuncAttributes fa{};
     if ((e = cudaFuncGetAttributes(&fa, fit64_kernel)) != cudaSuccess) return e;
     const int max_slice = (N + G - 1) / G + 1;
-    const long avail = (long)optin - (long)fa.sharedSizeBytes - 256;
+    const long avail = (long)optin - (long)fa.sharedSizeBytes;
     *rc = 0;
     *nbuf = 1;
     for (int r : {4, 2, 1})
@@ -242,6 +242,7 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
     a.upre = w.upre;
     a.partS = w.partS;
     a.LS = w.LS;
+    a.LA = w.LA;
     a.partA = w.partA;
     a.scal = w.scal;
     a.lam = w.lam;

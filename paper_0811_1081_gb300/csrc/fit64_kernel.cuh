@@ -18,7 +18,7 @@
 //     takes the start column R(k) of component k.
 // GB300 executes FP64 at 1/64 of its FP32 rate (2 FMAs per clock and SM), so the 2 M N
 // FMAs of a sweep bound this path: 4000 x 1500, 19 us at that rate; the sweep takes 29 and
-// the iteration 50 (122 in the form before: rows summed a warp each, sums over CTAs as one
+// the iteration 48 (122 in the form before: rows summed a warp each, sums over CTAs as one
 // thread's chain of 152 loads, roots and quotients in every thread).  So everything else is
 // arranged to cost few FP64 instructions and little latency: four rows share one
 // butterfly, a sum over CTAs is one round of loads of half a warp, one warp takes the
@@ -55,7 +55,8 @@ struct Fit64Args {
     double* upre;             // N: s' - W b' of the last iteration (pass scale)
     double* partS;            // G x LS: s' (or s0, column norms) partials, then the k-vector
     int LS;
-    double* partA;            // G x ldk: a' partials
+    double* partA;            // G x LA: a' partials
+    int LA;                   // ldk rounded up to a sector
     double* scal;             // G x 4: [0] ||v'||^2 / ||x||^2, [1] ||v' - V b'||^2, [2+b] ||ut[b]||^2
     double* lam;              // K
     int* iters;               // K
@@ -184,6 +185,48 @@ __device__ __forceinline__ void team_sums64(int G, int n, Src src, Stride stride
         if (sub == 0 && t < n) out(t, x);
     }
     __syncthreads();
+}
+
+// out(t) = the sum over the G CTAs of vec[t], t < n (`stride` doubles between CTAs, a multiple of
+// four).  All CTAs read the vector at the same time, so its few lines are what the L2 is
+// asked for: four neighbouring values (one sector) go to four lanes, the CTAs to the rest of
+// the warp and to the W warps that share four values; the warps' parts are added in order
+// through tmp (4 x kWarps64).  k = 10 and 152 CTAs: 2.2 us, 4.2 with team_sums64.  Ends with a CTA
+// barrier.
+template <class Out>
+__device__ __forceinline__ void team_vec64(int G, int n, const double* vec, size_t stride, double* tmp, Out out) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nq = (n + 3) / 4, W = nq < kWarps64 ? kWarps64 / nq : 1;
+    for (int unit = warp; unit < nq * W; unit += kWarps64) {
+        const int q = unit / W, p = unit % W, t = 4 * q + (lane & 3);
+        double x = 0.0;
+        if (t < n) {
+            const double* a = vec + t;
+#pragma unroll 5
+            for (int g = 8 * p + (lane >> 2); g < G; g += 8 * W) x += __ldcg(a + g * stride);
+        }
+        __syncwarp();
+        x += __shfl_xor_sync(kFull, x, 16);
+        x += __shfl_xor_sync(kFull, x, 8);
+        x += __shfl_xor_sync(kFull, x, 4);
+        if (W > 1) {
+            if (lane < 4) tmp[unit * 4 + lane] = x;
+        } else if (lane < 4 && t < n) {
+            out(t, x);
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    if (W > 1) {
+        if ((int)threadIdx.x < n) {
+            const int t = threadIdx.x;
+            const double* a = tmp + (t >> 2) * W * 4 + (t & 3);
+            double x = a[0];
+            for (int p = 1; p < W; ++p) x += a[4 * p];
+            out(t, x);
+        }
+        __syncthreads();
+    }
 }
 
 // Chunks of R on their way to shared memory: chunk q (counted on from sweep to sweep) is one
@@ -444,6 +487,7 @@ __global__ void __launch_bounds__(kBlock64, 1) fit64_kernel(const Fit64Args f) {
     extern __shared__ __align__(16) unsigned char dyn64[];
     __shared__ double red[kWarps64];
     __shared__ double sums[2];
+    __shared__ double team[4 * kWarps64];  // parts of a sum over the CTAs
     __shared__ double scal[4];  // lambda, 1 / ||u'||, 1 / ||v'||, the next loading's scale
     __shared__ int s_stop, s_dead;
     __shared__ uint64_t mbar[3];
@@ -472,7 +516,7 @@ __global__ void __launch_bounds__(kBlock64, 1) fit64_kernel(const Fit64Args f) {
     const double thresh = f.eps_thresh * sqrt(xx);
     if (tid == 0 && ldr > N) m.u[N] = 0.0;  // the padding column's loading
     double* pS = f.partS + (size_t)g * f.LS;
-    double* pA = f.partA + (size_t)g * f.ldk;
+    double* pA = f.partA + (size_t)g * f.LA;
     double* sc = f.scal + (size_t)g * 4;
     int status = kStOK, found = K;
     long long total = 0;
@@ -522,6 +566,9 @@ __global__ void __launch_bounds__(kBlock64, 1) fit64_kernel(const Fit64Args f) {
                 [&](int t) { return t < ns ? f.scal + (t == 0 ? 0 : slot) : t < ns + nc ? f.partS + n0 + t - ns : f.partS + N + t - ns - nc; },
                 [&](int t) { return t < ns ? (size_t)4 : (size_t)f.LS; },
                 [&](int t, double v) { (t < ns ? sums[t] : t < ns + nc ? m.sl[t - ns] : m.kb[t - ns - nc]) = v; });
+        };
+        auto gather_a = [&]() {
+            team_vec64(G, k, f.partA, (size_t)f.LA, team, [&](int t, double v) { m.ka[t] = v; });
         };
         gather_s(-1);
         double xxs = sums[0];
@@ -597,8 +644,7 @@ __global__ void __launch_bounds__(kBlock64, 1) fit64_kernel(const Fit64Args f) {
             // a = U_(k)^T s0 over the slice
             rows_t64(f.U, f.ldk, n0, n1, k, [&](int n) { return m.sl[n - n0]; }, pA, m.tmp);
             SYNC64();
-            team_sums64(G, k, [&](int t) { return f.partA + t; }, [&](int) { return (size_t)f.ldk; },
-                        [&](int t, double v) { m.ka[t] = v; });
+            gather_a();
         }
         {
             if (tid == 0) scal[0] = 1.0 / xxs;  // keeps the first loading's norm O(1)
@@ -736,8 +782,7 @@ __global__ void __launch_bounds__(kBlock64, 1) fit64_kernel(const Fit64Args f) {
             }
             if (gs && k > 0) {
                 if (!rows_norm) SYNC64();
-                team_sums64(G, k, [&](int t) { return f.partA + t; }, [&](int) { return (size_t)f.ldk; },
-                            [&](int t, double v) { m.ka[t] = v; });
+                gather_a();
             }
             fence_async_proxy();
             __syncthreads();

@@ -13,7 +13,7 @@ struct Workspace64 {
     double *R, *V, *U, *W, *vraw, *ut, *upre, *partS, *partA, *scal, *lam, *xpart, *cmean, *rmean;
     int *iters, *info, *abort, *lock;
     unsigned* flags;
-    int ld, LS, G;
+    int ld, LS, LA, G;
     size_t bytes;
 };
 
@@ -23,6 +23,7 @@ inline int ws64_ld(int K) { return (K + 1) / 2 * 2; }
 inline Workspace64 carve64_ws(void* base, long M, int N, int K, int G) {
     Workspace64 w{};
     w.ld = ws64_ld(K);
+    w.LA = (w.ld + 3) / 4 * 4;  // whole 32-byte sectors
     w.LS = N + w.ld;
     w.G = G;
     char* b = static_cast<char*>(base);
@@ -41,7 +42,7 @@ inline Workspace64 carve64_ws(void* base, long M, int N, int K, int G) {
     w.ut = (double*)take(sizeof(double) * 2 * (size_t)N);
     w.upre = (double*)take(sizeof(double) * (size_t)N);
     w.partS = (double*)take(sizeof(double) * (size_t)G * w.LS);
-    w.partA = (double*)take(sizeof(double) * (size_t)G * w.ld);
+    w.partA = (double*)take(sizeof(double) * (size_t)G * w.LA);
     w.scal = (double*)take(sizeof(double) * 4 * (size_t)G);
     w.lam = (double*)take(sizeof(double) * (size_t)K);
     w.xpart = (double*)take(sizeof(double) * kPack64Blocks);
