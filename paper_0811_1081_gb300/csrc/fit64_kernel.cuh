@@ -274,7 +274,8 @@ __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.
 // while the others add chunk t - 1 to the columns and chunk t + 1 is copied, so the FP64
 // pipe, which both share, is kept busy across the row sums' butterflies and the barriers
 // (29 us for 4000 x 1500, 34 with one after the other).  A chunk's four rows are summed
-// together by each of the eight warps over an eighth of the columns, and one butterfly reduces a lane's four sums (6 FP64 additions instead of 20).
+// together by each of the eight warps over an eighth of the columns, and one butterfly
+// reduces a lane's four sums (6 FP64 additions instead of 20).
 __device__ __forceinline__ double sweep64(const Fit64Args& f, const Smem64& m, Ring64& rg, double* red, int r0, int r1,
                                           bool start, bool deflate, double lamf, int kprev, int kcol) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x;
