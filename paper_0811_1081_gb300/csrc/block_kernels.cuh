@@ -224,7 +224,8 @@ __device__ __forceinline__ void jacobi_eig(JacobiMem& m, int n, bool vectors) {
     const int n2 = (n + 1) / 2 * 2, np = n2 / 2;  // an odd n plays with a dummy index n
     int cur = 0;
     if (vectors)
-        for (int e = t; e < kBlkMax * kBlkMax; e += kJacobiThreads) m.W[e % kBlkMax][e / kBlkMax] = e % kBlkMax == e / kBlkMax ? 1.0 : 0.0;
+        for (int e = t; e < kBlkMax * kBlkMax; e += kJacobiThreads)
+            m.W[e % kBlkMax][e / kBlkMax] = e % kBlkMax == e / kBlkMax ? 1.0 : 0.0;
     // an exact power of two brings the largest diagonal entry near 1, within FP32's range
     __syncthreads();
     double top = lane < n ? fabs(m.A[0][lane][lane]) : 0.0;

@@ -436,7 +436,8 @@ __device__ __forceinline__ double sweep64(const Fit64Args& f, const Smem64& m, R
 }
 
 // dst[j] = sum_{r in [a0, a1)} A[r * lda + j] y(r), j < kk.  `gw` lanes take
-// neighbouring columns, the warps and the rest of a warp share the rows; the parts are added in a fixed order through tmp (kWarps64 x 32).
+// neighbouring columns, the warps and the rest of a warp share the rows; the parts are added
+// in a fixed order through tmp (kWarps64 x 32).
 template <class Y>
 __device__ __forceinline__ void rows_t64(const double* A, int lda, int a0, int a1, int kk, Y y, double* dst,
                                          double* tmp) {
@@ -564,7 +565,10 @@ __global__ void __launch_bounds__(kBlock64, 1) fit64_kernel(const Fit64Args f) {
             const int ns = slot >= 0 ? 2 : 1;
             team_sums64(
                 G, ns + nc + nk,
-                [&](int t) { return t < ns ? f.scal + (t == 0 ? 0 : slot) : t < ns + nc ? f.partS + n0 + t - ns : f.partS + N + t - ns - nc; },
+                [&](int t) {
+                    if (t < ns) return f.scal + (t == 0 ? 0 : slot);
+                    return t < ns + nc ? f.partS + n0 + t - ns : f.partS + N + t - ns - nc;
+                },
                 [&](int t) { return t < ns ? (size_t)4 : (size_t)f.LS; },
                 [&](int t, double v) { (t < ns ? sums[t] : t < ns + nc ? m.sl[t - ns] : m.kb[t - ns - nc]) = v; });
         };
