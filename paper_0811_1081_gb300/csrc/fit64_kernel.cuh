@@ -524,6 +524,7 @@ __global__ void __launch_bounds__(kBlock64, 1) fit64_kernel(const Fit64Args f) {
     long long total = 0;
     bool alive = true;
     double lam_prev = 0.0, vinv_prev = 0.0, inv_nu = 0.0;
+    double gram_dev = 0.0, cut = 0.25;  // warp 0: ||V^T V - I||_F^2, and what b'^T b' / ||v'||^2 may reach
     int buf = 0;
 
 // Leaves the kernel when a copy of the sweep before did not arrive.
@@ -633,6 +634,18 @@ __global__ void __launch_bounds__(kBlock64, 1) fit64_kernel(const Fit64Args f) {
             xxs = sums[0];
         }
         if (gs && k > 0) {
+            // the Gram row is the new column of V^T V: how far V is from orthonormal bounds the error
+            // of ||v'||^2 - b'^T b' by ||V^T V - I||_F b'^T b' (NaN: cut is NaN, the rows are summed)
+            if (warp == 0) {
+                double e = 0.0;
+                for (int i = lane; i < k; i += 32) {
+                    const double d = i < k - 1 ? m.kb[i] : m.kb[i] - 1.0;
+                    e = fma(i < k - 1 ? 2.0 * d : d, d, e);
+                }
+                gram_dev += warp_sum(e);
+                const double dev = sqrt(gram_dev);
+                cut = dev <= 16.0 * DBL_EPSILON ? 0.25 : 4.0 * DBL_EPSILON / dev;
+            }
             // W <- R_k^T V for the deflation of component k-1: W(:, j) -= lambda u (v_{k-1} . v_j),
             // new column R_{k-1}^T v_{k-1} - lambda u |v_{k-1}|^2 with R_{k-1}^T v_{k-1} = u_pre / ||v' - V b'||
             const int km = k - 1;
@@ -723,15 +736,19 @@ __global__ void __launch_bounds__(kBlock64, 1) fit64_kernel(const Fit64Args f) {
                 }
                 __syncwarp();
             };
-            // V is orthonormal to FP64 rounding, so ||v' - V b'||^2 = ||v'||^2 - b'^T b'; the
-            // difference keeps its digits while b' is small (it is rounding after the deflation).
-            // Otherwise the norm is formed from the rows, with the second reduction.
+            // ||v' - V b'||^2 = ||v'||^2 - 2 b'^T b' + b'^T (V^T V) b', so with V orthonormal it is
+            // ||v'||^2 - b'^T b', which keeps its digits while b' is small: after the deflation b' is
+            // rounding where the earlier components have converged, and otherwise as large as what
+            // they are off (b'^T b' / ||v'||^2 of 0.4 with one iteration a component).  The difference is
+            // taken up to `cut`: 0.25, or less where V has lost orthonormality, so that the loss
+            // (V^T V - I enters with b'^T b') moves lambda by no more than three roundings.  Beyond,
+            // the norm is formed from the rows, with the second reduction.
             if (warp == 0) {
                 double bb = 0.0;
                 if (gs)
                     for (int i = lane; i < k; i += 32) bb = fma(m.kb[i], m.kb[i], bb);
                 bb = warp_sum(bb);
-                if (!gs || k == 0 || bb <= 0.25 * nvp) decide(nvp - bb);
+                if (!gs || k == 0 || bb <= cut * nvp) decide(nvp - bb);
                 else if (lane == 0) s_stop = -1;
                 __syncwarp();
             }
