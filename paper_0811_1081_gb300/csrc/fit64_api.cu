@@ -126,28 +126,14 @@ __global__ void unpack64_kernel(const double* R, int ldr, const double* V, const
     }
 }
 
-// Rows per staged chunk, chunks in shared memory and its bytes for rows of ldr doubles;
-// rc = 0 when even one row does not fit.  Three chunks (the sweep's pipeline) of four, two
-// or one rows where they fit (ldr up to about 2000, 3500, 5600), else one chunk of as many
-// rows as fit.
-cudaError_t plan64(int device, int ldr, int N, int ldk, int G, int* rc, int* nbuf, size_t* dyn) {
+// Chunks of the sweep for rows of ldr doubles (rc = 0 when even one row does not fit).
+cudaError_t plan64(int device, int ldr, int N, int ldk, int G, Chunks64* p) {
     int optin = 0;
     cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     if (e != cudaSuccess) return e;
     cudaFuncAttributes fa{};
     if ((e = cudaFuncGetAttributes(&fa, fit64_kernel)) != cudaSuccess) return e;
-    const int max_slice = (N + G - 1) / G + 1;
-    const long avail = (long)optin - (long)fa.sharedSizeBytes;
-    *rc = 0;
-    *nbuf = 1;
-    for (int r : {4, 2, 1})
-        if (*rc == 0 && (long)smem64_bytes(ldr, 3, r, ldk, max_slice) <= avail) {
-            *rc = r;
-            *nbuf = 3;
-        }
-    for (int r : {4, 3, 2, 1})
-        if (*rc == 0 && (long)smem64_bytes(ldr, 1, r, ldk, max_slice) <= avail) *rc = r;
-    *dyn = smem64_bytes(ldr, *nbuf, *rc > 0 ? *rc : 1, ldk, max_slice);
+    *p = plan_chunks64(ldr, ldk, (N + G - 1) / G + 1, (long)optin - (long)fa.sharedSizeBytes);
     return cudaSuccess;
 }
 
@@ -193,10 +179,10 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
     if (opts && opts->grid_ctas > 0 && opts->grid_ctas < G) G = opts->grid_ctas;
     const int ldk = w.ld;
     const int ldr = (N + 1) / 2 * 2;
-    int rc = 0, nbuf = 1;
-    size_t dyn = 0;
-    GS_CUDA(plan64(h->device, ldr, N, ldk, G, &rc, &nbuf, &dyn));
-    if (rc < 1) return GSPCA_ERR_NOT_SUPPORTED;
+    Chunks64 plan{};
+    GS_CUDA(plan64(h->device, ldr, N, ldk, G, &plan));
+    if (plan.rc < 1) return GSPCA_ERR_NOT_SUPPORTED;
+    const size_t dyn = plan.bytes;
     GS_CUDA(cudaFuncSetAttribute(fit64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
     int bps = 0;
     GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fit64_kernel, kBlock64, dyn));
@@ -252,8 +238,8 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
     a.abort = w.abort;
     a.iters_lock = lock_dev;
     a.timeout_ns = (unsigned long long)(timeout * 1e9);
-    a.rc = rc;
-    a.nbuf = nbuf;
+    a.rc = plan.rc;
+    a.nbuf = plan.nbuf;
     a.ldr = ldr;
     void* args[] = {&a};
     GS_CUDA(cudaEventRecord(h->ev0, s));

@@ -28,13 +28,9 @@
 #include <cfloat>
 
 #include "device_common.cuh"
+#include "plan64.cuh"
 
 namespace gspca {
-
-constexpr int kBlock64 = 512;
-constexpr int kWarps64 = kBlock64 / 32;
-constexpr int kMaxRc64 = 4;     // rows per staged chunk
-constexpr int kDotWarps64 = 8;  // warps that form the row sums of a chunk, two per scheduler
 
 struct Fit64Args {
     int M, N, K;
@@ -74,7 +70,6 @@ struct Fit64Args {
 // small vectors: row-sum parts (kMaxRc64 x kDotWarps64), row values and deflation weights
 // (2 x kMaxRc64 each), kb, ka (ldk), the slice (max N / G + 1).  rows_t64's scratch (kTmp64 doubles) is
 // the chunk memory, idle then, or follows where that is smaller.
-constexpr int kTmp64 = kWarps64 * 32;
 struct Smem64 {
     double* u;
     double* s;
@@ -110,13 +105,6 @@ __device__ __forceinline__ Smem64 carve64(unsigned char* dyn, const Fit64Args& f
     m.sl = p;
     m.tmp = f.nbuf * f.rc * f.ldr >= kTmp64 ? m.ch : p + max_slice;
     return m;
-}
-
-// Bytes of dynamic shared memory for rows of ldr doubles, nbuf chunks of rc rows, ldk, a slice.
-__host__ __device__ inline size_t smem64_bytes(int ldr, int nbuf, int rc, int ldk, int max_slice) {
-    const size_t chunk = (size_t)nbuf * rc * ldr;
-    return sizeof(double) * (2 * (size_t)ldr + chunk + kMaxRc64 * (kDotWarps64 + 4) + 2 * (size_t)ldk + max_slice +
-                             (chunk >= kTmp64 ? 0 : kTmp64));
 }
 
 // Lanes that share a row of kk values: the power of two that holds kk, at most 32.
