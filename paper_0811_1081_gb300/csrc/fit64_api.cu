@@ -127,13 +127,14 @@ __global__ void unpack64_kernel(const double* R, int ldr, const double* V, const
 }
 
 // Chunks of the sweep for rows of ldr doubles (rc = 0 when even one row does not fit).
-cudaError_t plan64(int device, int ldr, int N, int ldk, int G, Chunks64* p) {
+cudaError_t plan64(int device, int ldr, int M, int N, int ldk, int G, Chunks64* p) {
     int optin = 0;
     cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     if (e != cudaSuccess) return e;
     cudaFuncAttributes fa{};
-    if ((e = cudaFuncGetAttributes(&fa, fit64_kernel)) != cudaSuccess) return e;
-    *p = plan_chunks64(ldr, ldk, (N + G - 1) / G + 1, (long)optin - (long)fa.sharedSizeBytes);
+    if ((e = cudaFuncGetAttributes(&fa, ldr <= kShortLdr64 ? fit64_kernel<true> : fit64_kernel<false>)) != cudaSuccess)
+        return e;
+    *p = plan_chunks64((M + G - 1) / G, ldr, ldk, (N + G - 1) / G + 1, (long)optin - (long)fa.sharedSizeBytes);
     return cudaSuccess;
 }
 
@@ -180,12 +181,13 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
     const int ldk = w.ld;
     const int ldr = (N + 1) / 2 * 2;
     Chunks64 plan{};
-    GS_CUDA(plan64(h->device, ldr, N, ldk, G, &plan));
+    GS_CUDA(plan64(h->device, ldr, M, N, ldk, G, &plan));
     if (plan.rc < 1) return GSPCA_ERR_NOT_SUPPORTED;
     const size_t dyn = plan.bytes;
-    GS_CUDA(cudaFuncSetAttribute(fit64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    const auto fit64 = plan.rc == kShortRc64 ? fit64_kernel<true> : fit64_kernel<false>;
+    GS_CUDA(cudaFuncSetAttribute(fit64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
     int bps = 0;
-    GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fit64_kernel, kBlock64, dyn));
+    GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fit64, kBlock64, dyn));
     if (bps < 1) return GSPCA_ERR_NOT_SUPPORTED;
 
     const int center = opts ? opts->center : 0;
@@ -243,7 +245,7 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
     a.ldr = ldr;
     void* args[] = {&a};
     GS_CUDA(cudaEventRecord(h->ev0, s));
-    GS_CUDA(cudaLaunchCooperativeKernel((const void*)fit64_kernel, dim3(G), dim3(kBlock64), args, dyn, s));
+    GS_CUDA(cudaLaunchCooperativeKernel((const void*)fit64, dim3(G), dim3(kBlock64), args, dyn, s));
     ++launches;
     GS_CUDA(cudaEventRecord(h->ev1, s));
     epilogue64_kernel<<<256, 256, 0, s>>>(w.V, w.U, ldk, w.lam, w.iters, w.info, M, N, K, algo == GSPCA_GS,

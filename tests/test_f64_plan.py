@@ -17,10 +17,10 @@ PROBE = r"""
 #include "plan64.cuh"
 using namespace gspca;
 int main() {
-    int ldr, ldk, slice;
+    int rows, ldr, ldk, slice;
     long avail;
-    while (std::scanf("%d %d %d %ld", &ldr, &ldk, &slice, &avail) == 4) {
-        const Chunks64 p = plan_chunks64(ldr, ldk, slice, avail);
+    while (std::scanf("%d %d %d %d %ld", &rows, &ldr, &ldk, &slice, &avail) == 5) {
+        const Chunks64 p = plan_chunks64(rows, ldr, ldk, slice, avail);
         std::printf("%d %d %zu %zu %zu\n", p.rc, p.nbuf, p.bytes, smem64_bytes(ldr, 1, 1, ldk, slice),
                     smem64_bytes(ldr, p.nbuf, p.rc + 1, ldk, slice));
     }
@@ -35,9 +35,9 @@ def plan(tmp_path_factory):
     src.write_text(PROBE)
     subprocess.run(["g++", "-std=c++17", "-Wall", "-Werror", "-I", CSRC, str(src), "-o", str(exe)], check=True)
 
-    def run(shapes):
-        """[(N, K, G)] -> [(rows per chunk, chunks, bytes, bytes of one row, bytes of one row more)]"""
-        lines = ["%d %d %d %d" % ((n + 1) // 2 * 2, (k + 1) // 2 * 2, (n + g - 1) // g + 1, OPTIN - STATIC)
+    def run(shapes, rows=20):
+        """[(N, K, G)], the rows of a CTA -> [(rows per chunk, chunks, bytes, bytes of one row, bytes of one row more)]"""
+        lines = ["%d %d %d %d %d" % (rows, (n + 1) // 2 * 2, (k + 1) // 2 * 2, (n + g - 1) // g + 1, OPTIN - STATIC)
                  for n, k, g in shapes]
         out = subprocess.run([str(exe)], input="\n".join(lines), capture_output=True, text=True, check=True).stdout
         return [tuple(int(x) for x in line.split()) for line in out.splitlines()]
@@ -62,3 +62,13 @@ def test_every_column_count_fits(plan):
     """Up to 8192 columns with K to 300: at least one row per chunk (K a little less where one CTA owns every column)."""
     shapes = [(n, k, 152) for n in range(300, 8193, 131) for k in (2, 300)]
     assert all(p[0] >= 1 for p in plan(shapes + [(8192, 300, 152), (8192, 2, 8)]))
+
+
+def test_short_rows_share_a_stage(plan):
+    """Rows of up to 256 doubles are staged 32 at a time, whatever K and the grid, unless a CTA has at
+    most eight; longer ones at most four."""
+    shapes = [(n, k, g) for n in [1, 2, 3, 31, 60, 129, 255, 256] for k in {1, min(n, 34), n} for g in [1, 2, 152]]
+    for s, (rc, nbuf, used, _, _), few in zip(shapes, plan(shapes, rows=9), plan(shapes, rows=8)):
+        assert (rc, nbuf) == (32, 3) and used <= OPTIN - STATIC, s
+        assert few[:2] == (4, 3), s
+    assert all(p[0] == 4 for p in plan([(257, 5, 152), (258, 257, 1), (1500, 50, 152)]))
