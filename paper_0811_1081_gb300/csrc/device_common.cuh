@@ -157,6 +157,23 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// Warp sums of four values per lane in one butterfly: lanes 8 q to 8 q + 7 return value q's, the
+// pairs added in warp_sum's order.
+__device__ __forceinline__ double warp_sum4(const double (&a)[4]) {
+    const int lane = threadIdx.x & 31;
+    // lanes >= 16 keep values 2, 3, then lanes with bit 3 the odd ones
+    const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0;
+    double x = h16 ? a[2] : a[0], y = h16 ? a[3] : a[1];
+    x += __shfl_xor_sync(kFull, h16 ? a[0] : a[2], 16);
+    y += __shfl_xor_sync(kFull, h16 ? a[1] : a[3], 16);
+    double t = h8 ? y : x;
+    t += __shfl_xor_sync(kFull, h8 ? x : y, 8);
+    t += __shfl_xor_sync(kFull, t, 4);
+    t += __shfl_xor_sync(kFull, t, 2);
+    t += __shfl_xor_sync(kFull, t, 1);
+    return t;
+}
+
 // Reduce V independent per-lane values over the 32 lanes with a butterfly that
 // halves the live values at every level: log2(V) exchange levels move V-1
 // values in total, then 5-log2(V) plain levels finish the sum.  On return

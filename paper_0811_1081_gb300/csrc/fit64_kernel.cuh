@@ -260,22 +260,6 @@ struct Ring64 {
 
 __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
-// Warp sums of four rows' lane values in one butterfly: lanes 8 q to 8 q + 7 return row q's.
-__device__ __forceinline__ double rows4_sum(const double (&a)[4]) {
-    const int lane = threadIdx.x & 31;
-    // lanes >= 16 keep rows 2, 3, then lanes with bit 3 the odd ones
-    const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0;
-    double x = h16 ? a[2] : a[0], y = h16 ? a[3] : a[1];
-    x += __shfl_xor_sync(kFull, h16 ? a[0] : a[2], 16);
-    y += __shfl_xor_sync(kFull, h16 ? a[1] : a[3], 16);
-    double t = h8 ? y : x;
-    t += __shfl_xor_sync(kFull, h8 ? x : y, 8);
-    t += __shfl_xor_sync(kFull, t, 4);
-    t += __shfl_xor_sync(kFull, t, 2);
-    t += __shfl_xor_sync(kFull, t, 1);
-    return t;
-}
-
 // One sweep over the CTA's rows [r0, r1).
 //   start == false: row value x_r = R_r . u (u in smem), written to vraw;
 //   start == true:  with `deflate`, R_r <- R_r - a_r u^T first (a_r = lamf V[r, kprev],
@@ -367,7 +351,7 @@ __device__ __forceinline__ double sweep64(const Fit64Args& f, const Smem64& m, R
                     }
             }
         }
-        const double t = rows4_sum(a);
+        const double t = warp_sum4(a);
         if ((lane & 7) == 0 && (lane >> 3) < nr) m.part[(lane >> 3) * kDotWarps64 + warp] = t;
         __syncwarp();
         asm volatile("barrier.sync 1, %0;" ::"n"(32 * kDotWarps64) : "memory");
@@ -498,7 +482,7 @@ __device__ __forceinline__ double sweep64_short(const Fit64Args& f, const Smem64
             }
         }
         __syncwarp();
-        const double v = rows4_sum(a);
+        const double v = warp_sum4(a);
         const int r = 4 * warp + (lane >> 3);
         if ((lane & 7) == 0 && r < nr) {
             rowv[r] = v;

@@ -295,23 +295,37 @@ inline FitArgs make_args(const Workspace& w, const Plan& p, int M, int N, int K,
     return a;
 }
 
-// Column means of X into w.cmean; the chunk sums go where the fit's pass partials will
-// (w.G x w.LA floats).  Returns the kernels launched.
+// Column means of X into w.cmean.  Returns the kernels launched.
+// The form and the chunks follow from the layout, M and N alone, so every entry point adds in the
+// same order; the chunk sums go where the pack kernel will write R (8 N bytes per 64 rows or more
+// of 4 N bytes each).
+// One launch, a warp per column, while its M / 32 dependent steps (0.14 us each) cost less than the
+// second launch and the blocks' sums (rows x columns, us, one launch / chunks):
+//   column-major 300 x 60 6.3 / 10, 300 x 1000 6.4 / 13, 1500 x 700 13 / 17, 2000 x 1000 15 / 23,
+//   5000 x 1000 29 / 33, 10000 x 2000 96 / 106, 20000 x 2000 185 / 193, 300 x 7500 27 / 25 (but 147 / 157
+//   in the whole call); row-major 300 x 60 6.5 / 8.5, 300 x 1000 8.3 / 12, 2000 x 1000 15 / 19,
+//   5000 x 1000 29 / 29, 10000 x 2000 97 / 99;
+// chunks beyond: column-major 2000 x 100 15 / 11, 5000 x 500 29 / 25, 1000 x 7500 64 / 41, 30000 x 1000
+//   144 / 130; row-major 2000 x 100 15 / 11, 5000 x 500 29 / 23, 300 x 7500 27 / 17.
+// 608 blocks are four per SM of 152 (100000 x 130 row-major: 100, 88 and 87 us with 304, 608 and
+// 1216; 5000 x 1000: 37, 29 and 31), chunks of at least 64 rows (300 x 60: 8.5 us, 10 and 13 with 128
+// and 256) and at most 128 of them (100000 x 130: 121, 95, 88 and 88 us with 32, 64, 128 and 256;
+// 1000000 x 8 column-major: 156 with 64, 93 with 128).
 inline int enqueue_colmean(const Workspace& w, cudaStream_t s, const float* X, gspca_layout layout, long ldx, int M,
                            int N) {
-    const int gx = (N + 31) / 32;
-    const size_t room = sizeof(float) * (size_t)w.G * w.LA / (sizeof(double) * (size_t)N);
-    int chunks = (608 + gx - 1) / gx;  // four blocks per SM
-    if (chunks > 64) chunks = 64;
-    if ((size_t)chunks > room) chunks = (int)room;
-    if (chunks < 2) {
+    const bool col = layout == GSPCA_COL_MAJOR;
+    const int fills = col && N >= 1000 ? 20000 : 2048;
+    if (M <= 64 || (col && M <= 512) || (N <= 2048 && (M <= 512 || (N >= 512 && M <= fills)))) {
         colmean_kernel<<<(N + 7) / 8, 256, 0, s>>>(X, (int)layout, ldx, M, N, w.cmean);
         return 1;
     }
+    const int gx = (N + 31) / 32;
+    int chunks = (608 + gx - 1) / gx;
+    if (chunks > 128) chunks = 128;
     int rows_per = (M + chunks - 1) / chunks;
     if (rows_per < 64) rows_per = 64;
     chunks = (M + rows_per - 1) / rows_per;
-    double* part = reinterpret_cast<double*>(w.partA);
+    double* part = reinterpret_cast<double*>(w.R);
     colmean_part_kernel<<<dim3(gx, chunks), 256, 0, s>>>(X, (int)layout, ldx, M, N, rows_per, part);
     colmean_sum_kernel<<<(N + 127) / 128, 128, 0, s>>>(part, chunks, M, N, w.cmean);
     return 2;

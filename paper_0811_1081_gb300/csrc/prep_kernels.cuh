@@ -13,7 +13,8 @@ __device__ __forceinline__ float load_x(const float* X, int layout, long ldx, in
     return layout == 0 ? X[(size_t)c * ldx + r] : X[(size_t)r * ldx + c];
 }
 
-// mean over rows of every column (warp per column), FP64 sums.
+// mean over rows of every column (warp per column), FP64 sums: one launch, for small matrices and
+// where the columns alone fill the chip (enqueue_colmean has the line and both sides).
 static __global__ void colmean_kernel(const float* X, int layout, long ldx, int M, int N, double* mean) {
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -24,27 +25,37 @@ static __global__ void colmean_kernel(const float* X, int layout, long ldx, int 
     if (lane == 0) mean[c] = s / (double)M;
 }
 
-// Column means in two steps, FP64 sums: a block adds a chunk of rows of 32 columns
-// (8 row lanes, combined in lane order) into part[chunk][c]; then a thread per
-// column adds the chunks in order.  Reads are coalesced in both layouts; a warp
-// per column (colmean_kernel, kept where there is no scratch for the chunk sums) leaves
-// most of the chip idle on narrow matrices and strides through row-major ones
-// (60001 x 130 row-major, centred fit with 8 components: 5.00 ms, 4.72 this way).
+// Column means in two steps, FP64 sums: a block adds a chunk of rows of 32 columns into
+// part[chunk][c] (row-major: 8 row lanes, combined in lane order; column-major: a warp takes four
+// columns at once, lanes along the rows, one butterfly for the four); then a thread per
+// column adds the chunks in order.  Reads are coalesced in both layouts and narrow matrices fill
+// the chip; bound by the FP64 pipe (a conversion and an addition per element: 64 us for 10000 x
+// 2000).  60001 x 130: 62 us row-major, 61 column-major, a warp per column 270 and 271.
 static __global__ void __launch_bounds__(256) colmean_part_kernel(const float* __restrict__ X, int layout, long ldx,
                                                                   int M, int N, int rows_per, double* part) {
     __shared__ double acc[8][33];
     const int t = threadIdx.x, c0 = blockIdx.x * 32;
     const int ra = blockIdx.y * rows_per, rb = min(M, ra + rows_per);
-    if (layout == 0) {  // a warp takes 4 columns, lanes along the rows
-        const int lane = t & 31, warp = t >> 5;
-        for (int q = 0; q < 4; ++q) {
-            const int c = c0 + warp * 4 + q;
-            double s = 0.0;
-            if (c < N)
-                for (int r = ra + lane; r < rb; r += 32) s += (double)X[(size_t)c * ldx + r];
-            s = warp_sum(s);
-            if (lane == 0 && c < N) part[(size_t)blockIdx.y * N + c] = s;
+    if (layout == 0) {
+        const int lane = t & 31, cw = c0 + (t >> 5) * 4, nc = min(4, N - cw);
+        if (nc <= 0) return;
+        const float* p = X + (size_t)cw * ldx;
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+        if (nc == 4) {
+#pragma unroll 2
+            for (int r = ra + lane; r < rb; r += 32)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) s[q] += (double)p[(size_t)q * ldx + r];
+        } else {
+            for (int r = ra + lane; r < rb; r += 32)
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if (q < nc) s[q] += (double)p[(size_t)q * ldx + r];
         }
+        __syncwarp();
+        const double v = warp_sum4(s);
+        const int q = lane >> 3;
+        if ((lane & 7) == 0 && q < nc) part[(size_t)blockIdx.y * N + cw + q] = v;
     } else {
         const int cc = t & 31, ty = t >> 5, c = c0 + cc;
         double s = 0.0;
