@@ -274,13 +274,15 @@ extern "C" gspca_status gspca_fit_f64(gspca_t h, void* stream, const double* X, 
     const int st = h->h_info[0];
     h->last.found = h->h_info[1];
     h->last.total_iters = (long long)h->h_info[2] + ((long long)h->h_info[3] << 31);
-    // algorithmic bytes: one FP64 read of R per sweep, the deflation's write per component,
-    // GS factor reads (V twice, W, U twice per iteration)
+    // algorithmic bytes: one FP64 read of R per sweep, the deflation's write per component, GS factor
+    // reads: V once per iteration (b') and at a component's end (its new column), W once, U twice
+    // per iteration (a' and the next loading; the last iteration's two are the component's
+    // start's).  Iterations that sum the rows for the norm read V once more, not counted.
     double b = 0.0;
     const double mn = 8.0 * M * N;
     for (int k = 0; k < h->last.found; ++k) {
         b += ((double)hiters[k] + 1.0) * mn + (k > 0 ? mn : 0.0);
-        if (algo == GSPCA_GS && k > 0) b += (double)hiters[k] * (2.0 * M * k + 3.0 * N * k) * 8.0;
+        if (algo == GSPCA_GS && k > 0) b += (((double)hiters[k] + 1.0) * M * k + 3.0 * hiters[k] * N * k) * 8.0;
     }
     h->last.alg_bytes = b;
     if (st == kStDegenerate) return GSPCA_ERR_DEGENERATE;
