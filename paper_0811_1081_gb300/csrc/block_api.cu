@@ -299,7 +299,7 @@ extern "C" gspca_status gspca_fit_block(gspca_t h, void* stream, const float* X,
     h->last.kernel_launches = launches;
     h->last.grid_ctas = kGramCtas;
     h->last.team_ctas = 0;
-    h->last.block_threads = 1024;
+    h->last.block_threads = kGramThreads;
     h->last.batch_pass = 0;
     // algorithmic bytes: per iteration R read twice (R U, R^T V) and the factors of the earlier
     // blocks twice on each side (projections); per block R read and written once (deflation)

@@ -19,3 +19,18 @@ def test_f64_algorithmic_bytes(gp, algo):  # noqa: F811
     if algo == "gs":
         want += sum((it + 1) * M * k + 3 * it * N * k for k, it in enumerate(lock))
     assert b == 8 * want
+
+
+def test_block_launch_shape(gp):  # noqa: F811
+    """A block fit reports the Gram kernel's launch, grid and block."""
+    import os
+    import re
+
+    import torch
+
+    src = open(os.path.join(os.path.dirname(gp.__file__), "csrc", "block_kernels.cuh")).read()
+    const = {n: int(v) for n, v in re.findall(r"constexpr int (kGram\w+) = (\d+);", src)}
+    X = torch.from_numpy(np.random.default_rng(2).standard_normal((300, 60)).astype(np.float32)).cuda()
+    with gp.Handle(300, 60, 4) as h:
+        info = h.fit_block(X, 4, block=2, tol=1e-3, max_iter=5).info
+    assert (info["grid_ctas"], info["block_threads"]) == (const["kGramCtas"], const["kGramThreads"])
