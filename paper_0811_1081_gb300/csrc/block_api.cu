@@ -209,20 +209,22 @@ extern "C" gspca_status gspca_fit_block(gspca_t h, void* stream, const float* X,
         };
         if (half_step(w.U, w.V, w.flag) != GSPCA_OK) return GSPCA_ERR_CUDA;
         int j = 0, fl = 0;
+        double change = 1.0, before = 1.0;  // of the Ritz values, in the last test and the one before
         bool last = false;
         for (;;) {
             // Z = R^T V, against U_(k0); Ritz values from Z^T Z
             BL_CUBLAS(cublasSgemm(cb, CUBLAS_OP_T, CUBLAS_OP_N, N, bw, M, &one, R, M, w.V, M, &zero, w.Z, N));
             if (project_out(cb, P, N, k0, w.Z, bw, w.tmp) != GSPCA_OK) return GSPCA_ERR_CUDA;
             gram(s, w.Z, N, w.Z, N, N, bw, bw, w.partZ);
-            // The test, one CTA and a long chain, runs on a stream of its own.  The next U = qr(Z) and
-            // V = qr(R U) go ahead meanwhile, into second buffers and with the other flag word, and
-            // are dropped when the test says stop: 10000 x 2000, two blocks of 16, 6 iterations each,
-            // 6.1 ms with the test before them, 4.8 so.  Not where this iteration is the last in any
-            // case.
+            // The test, one CTA and a long chain, runs on a stream of its own, and the next U = qr(Z) and
+            // V = qr(R U) go ahead meanwhile, into second buffers and with the other flag word:
+            // 10000 x 2000, two blocks of 16, 6 iterations each, 6.1 ms with the test before them, 4.8 so.
+            // They are dropped when the test says stop, and left out where this iteration is the last
+            // in any case.
             GS_CUDA(cudaEventRecord(h->blk_gram, s));
             GS_CUDA(cudaStreamWaitEvent(h->blk_stream, h->blk_gram, 0));
-            ritz_test_kernel<<<1, kJacobiThreads, 0, h->blk_stream>>>(w.partZ, w.sp, bw, tol, w.flag + (j & 1), h->h_blk);
+            ritz_test_kernel<<<1, kJacobiThreads, 0, h->blk_stream>>>(w.partZ, w.sp, bw, tol, w.flag + (j & 1), h->h_blk,
+                                                                    reinterpret_cast<float*>(h->h_blk + 2));
             GS_CUDA(cudaGetLastError());
             GS_CUDA(cudaEventRecord(h->blk_test, h->blk_stream));
             launches += 3 + (k0 > 0 ? 2 : 0);
@@ -230,12 +232,35 @@ extern "C" gspca_status gspca_fit_block(gspca_t h, void* stream, const float* X,
             ++total;
             last = opts && opts->iters_lock ? j >= opts->iters_lock[k0] : j >= max_iter;
             if (last) break;
+            // Where the test is likely to stop the block they wait for it: the first test compares with
+            // zero, a change of 1, so it stops a block exactly when tol > 1; later changes shrink
+            // about as the one before did (to a tenth where nothing is known).  Only narrow blocks go
+            // by that guess: their test is short (a wrong guess costs one) and the half step is not;
+            // a wide block's test hides all or most of it, and a wrong guess would cost 0.14 (16) to
+            // 0.45 ms (32).  15000 x 7500, two blocks of 1: 3.58 ms with tol 10, 3.24 so, 9.98 and 9.62
+            // with 1e-3; 10000 x 2000, blocks of 4, 1e-2: 2.72 and 2.61.
+            const bool locked = opts && opts->iters_lock;
+            const double guess = j == 1 ? 1.0 : change * change / before;
+            const bool ahead = locked || guess >= tol || (j > 1 && bw > 4);
+            const auto tested = [&]() -> cudaError_t {
+                const cudaError_t e = cudaEventSynchronize(h->blk_test);
+                fl = ((volatile int*)h->h_blk)[0];
+                before = j == 1 ? 10.0 : change;
+                change = ((volatile float*)h->h_blk)[2];
+                return e;
+            };
+            const auto ends = [&] { return (fl & 1) || (!locked && (fl & 2)); };  // dependent columns, or stop
             int* nflag = w.flag + (j & 1);
+            if (!ahead) {
+                GS_CUDA(tested());
+                if (ends()) break;
+            }
             if (cholqr2(cb, s, w.Z, w.Unext, N, bw, w, w.partZ, nflag, &launches) != GSPCA_OK) return GSPCA_ERR_CUDA;
             if (half_step(w.Unext, w.Vnext, nflag) != GSPCA_OK) return GSPCA_ERR_CUDA;
-            GS_CUDA(cudaEventSynchronize(h->blk_test));
-            fl = ((volatile int*)h->h_blk)[0];
-            if ((fl & 1) || (!(opts && opts->iters_lock) && (fl & 2))) break;  // dependent columns, or stop
+            if (ahead) {
+                GS_CUDA(tested());
+                if (ends()) break;
+            }
             std::swap(w.U, w.Unext);
             std::swap(w.V, w.Vnext);
         }

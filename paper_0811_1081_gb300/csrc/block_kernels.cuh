@@ -329,9 +329,11 @@ __device__ __forceinline__ void jacobi_eig(JacobiMem& m, int n, bool vectors) {
 
 // Ritz values s_i = sqrt(max(ev_i, 0)) of the Gram matrix Z^T Z (given as parts), in
 // decreasing order; the block stops when every |s_i - sp_i| < tol s_i; then sp <- s.  The
-// host reads *host = *flag | 2 (stop); *flag is cleared for the iteration after the next.  One CTA.
+// host reads *host = *flag | 2 (stop) and *change = the largest |s_i - sp_i| / s_i in FP32, by which
+// it guesses the next test; *flag is cleared for the iteration after the next.  One CTA.
 __global__ void __launch_bounds__(kJacobiThreads) ritz_test_kernel(const double* part, double* sp, int n, double tol,
-                                                                   int* flag, volatile int* host) {
+                                                                   int* flag, volatile int* host,
+                                                                   volatile float* change) {
     __shared__ JacobiMem m;
     const int t = threadIdx.x;
     for (int e = t; e < kBlkMax * (kBlkMax + 1); e += kJacobiThreads) (&m.A[0][0][0])[e] = 0.0;
@@ -340,13 +342,18 @@ __global__ void __launch_bounds__(kJacobiThreads) ritz_test_kernel(const double*
     __syncthreads();
     jacobi_eig(m, n, false);
     bool same = true;
+    float rel = 0.f;
     if (t < n) {
-        const double ev = m.ev[t], s = sqrt(ev > 0.0 ? ev : 0.0);
-        same = fabs(sp[m.rank[t]] - s) < tol * s;
+        const double ev = m.ev[t], s = sqrt(ev > 0.0 ? ev : 0.0), d = fabs(sp[m.rank[t]] - s);
+        same = d < tol * s;
+        rel = (float)d / (float)s;
         sp[m.rank[t]] = s;
     }
+    static_assert(kBlkMax == 32, "a warp holds the values");
+    for (int o = 16; o >= 1; o >>= 1) rel = fmaxf(rel, __shfl_xor_sync(kFull, rel, o));
     const int stop = __syncthreads_and(same);
     if (t == 0) {
+        *change = rel;
         *host = *flag | (stop ? 2 : 0);
         *flag = 0;
     }
