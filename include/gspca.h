@@ -244,7 +244,10 @@ gspca_status gspca_fit_f64(gspca_t h, void *stream, const double *X, gspca_layou
  * coef_trace give GSPCA_ERR_NOT_SUPPORTED).  A block whose start or iterate has
  * numerically dependent columns ends the fit with GSPCA_ERR_DEGENERATE (earlier
  * blocks kept).  The first call on a handle allocates the block workspace and a
- * cuBLAS handle (owned by the handle).  Synchronises `stream` once per iteration. */
+ * cuBLAS handle, a stream and two events (owned by the handle; the convergence test
+ * runs on that stream).  The host waits for the test once per iteration, in general
+ * with the next half step already queued on `stream`, and for `stream` itself at
+ * the end of a block and of the call. */
 gspca_status gspca_fit_block(gspca_t h, void *stream, const float *X, gspca_layout layout, long ldx, int M, int N,
                              int K, int block, double tol, int max_iter, float *T, float *P, double *lambda,
                              int *iters, float *R_out, const gspca_opts *opts);
