@@ -215,7 +215,9 @@ struct JacobiMem {
 // `vectors` the unit vectors are the columns of m.W.  One CTA.
 // A step is a chain of two barriers, the rotation and its use, so the rotation is kept short:
 // the tangent comes from FP32 (its error leaves 1e-7 of an entry, removed with what the next
-// sweep removes anyway), the cosine from it in FP64, so rotations are orthogonal to FP64.  A
+// sweep removes anyway), the cosine from it in FP64, so rotations are orthogonal to FP64 (n = 8,
+// 11, 16, 24 matrices of each of three spectra against 40 digits: the errors of eigenvalues and
+// vectors are those of FP64 tangents to 0.9 to 1.2 in the mean, with as many sweeps).  A
 // thread takes a column of a 2 x 2 block through both sides at once, from one copy of the
 // matrix into the other.  n = 16: 142 us; 445 with four barriers a step, FP64 quotients and
 // roots, and the norms and the order found by one thread.
